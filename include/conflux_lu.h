@@ -321,7 +321,7 @@ typedef struct {
     int krylov_products;    /* products A z inside FGMRES: 0 (default) binary32
                                accuracy first, binary64 from the first cycle
                                that cuts eta by less than 10x; 1 binary64
-                               only; 2 binary32 accuracy only                 */
+                               accuracy only; 2 binary32 accuracy only        */
     int inner_steps;        /* binary32-product inner steps per classical step
                                (0: default 3; negative: none)                  */
     int reserved[2];        /* must be zero                                     */
@@ -355,7 +355,7 @@ typedef struct {
  * 2x or falls below 1e-6 |r|), then x += d.  After that the correction equation is
  * solved by right-preconditioned flexible GMRES (binary64 Arnoldi and
  * Gram-Schmidt, the fp32 LU solve as preconditioner).  Its products A z
- * are first computed in binary32 accuracy (exact sums of four 8-bit digits of
+ * are first computed in binary32 accuracy (exact sums of five 8-bit digits of
  * A and z; below 256 rows binary32 multiplies) with an inner tolerance of 1e-6: the
  * outer binary64 residual corrects what they miss.  Once such a cycle cuts
  * eta by less than 10x the products are binary64 (kappa too large for
