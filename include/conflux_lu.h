@@ -252,7 +252,7 @@ int lu_residual(int n, int nrhs, const double *A, int lda, const double *X,
  * allocator owns the GPU's memory.  The paper has no counterpart; this is a
  * deployment variant of the residual and backward-error computation.
  *
- * Same arguments, results and layouts as lu_residual, with nrhs <= 64
+ * Same arguments, results (bit for bit) and layouts as lu_residual, with nrhs <= 64
  * (larger nrhs returns -2 before any work).  It calls no cudaMalloc,
  * cudaFree or other allocating routine.  Its reduction scratch is one fixed
  * array of about 160 KB per device, placed in the library and kept until the

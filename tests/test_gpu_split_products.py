@@ -69,3 +69,25 @@ def test_a_row_is_the_same_beside_other_rows(kind):
     A2[1::2] = np.ldexp(A2[1::2], (np.arange(320) * 11 % 90 - 45)[None, :])
     A2[3, 70], A2[5, 200] = np.inf, np.nan
     np.testing.assert_array_equal(_residual(A2, X, B)[::2], R[::2])
+
+
+@pytest.mark.parametrize("n,nrhs", [(255, 16), (256, 1), (257, 17), (333, 16), (1000, 33), (2500, 64)])
+@pytest.mark.parametrize("kind", ["normal", "plain10", "diagonal"])
+def test_the_form_without_workspace_has_the_same_bits(n, nrhs, kind):
+    """What a call returns does not depend on whether its workspace was to be
+    had: lu_residual_noalloc has none.  One and several splits of the columns,
+    a last split that is short, rows and columns off the tiles, unaligned rows."""
+    torch = cuda_or_fail()
+    lib()
+    from paper_2010_05975_gb300 import _native as nat
+    L = nat.library()
+    A, X, B = (torch.from_numpy(M.copy()).cuda() for M in _data(n, nrhs, kind))
+    out = []
+    for fn in (L.lu_residual, L.lu_residual_noalloc):
+        R = torch.full((n, nrhs), float("nan"), dtype=torch.float64, device="cuda")
+        eta = torch.full((nrhs,), float("nan"), dtype=torch.float64, device="cuda")
+        assert fn(n, nrhs, A.data_ptr(), n, X.data_ptr(), nrhs, B.data_ptr(), nrhs, R.data_ptr(), nrhs,
+                  eta.data_ptr(), torch.cuda.current_stream().cuda_stream) == 0
+        out.append((R.cpu().numpy(), eta.cpu().numpy()))
+    np.testing.assert_array_equal(out[0][0].view(np.int64), out[1][0].view(np.int64))
+    np.testing.assert_array_equal(out[0][1], out[1][1])
