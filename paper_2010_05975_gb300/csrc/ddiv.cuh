@@ -1,10 +1,8 @@
 // Correctly rounded binary64 division in 32-bit integer arithmetic.
 //
 // GB300 executes every binary64 instruction of a warp in 64 cycles of its
-// scheduler's one FP64 pipe, whatever the number of active lanes, and the
-// hardware division is nine of them in a row: 565 cycles of latency (1 096 for
-// two warps of one scheduler), during which no other binary64 work runs
-// there.  The panel kernels divide once per row and column on their critical
+// scheduler's one FP64 pipe, whatever the number of active lanes, and a
+// division takes 565 cycles (1 096 for two warps of one scheduler).  The panel kernels divide once per row and column on their critical
 // path.  The schoolbook division below needs about 70 integer instructions
 // and no FP64 pipe.
 //
@@ -30,15 +28,43 @@
 
 namespace lu {
 
+#ifdef __CUDACC__                                  // (a host build brings its own)
+__device__ __forceinline__ float approx_rcp(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float approx_rsqrt(float x) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+// volatile: not computed ahead of the branch that needs them
+__device__ __forceinline__ double hardware_div(double a, double b) {
+    double r;
+    asm volatile("div.rn.f64 %0, %1, %2;" : "=d"(r) : "d"(a), "d"(b));
+    return r;
+}
+__device__ __forceinline__ double hardware_sqrt(double x) {
+    double r;
+    asm volatile("sqrt.rn.f64 %0, %1;" : "=d"(r) : "d"(x));
+    return r;
+}
+#endif
+
+// An approximation of a value in [1/2, 1] as an integer in units of 2^-32.
+// (Approximations may come out below 1/2 or above 1.)
+__device__ __forceinline__ unsigned approx_bits(float y) {
+    const unsigned b = __float_as_uint(y);
+    return b >= 0x3f800000u ? 0xffffffffu : b < 0x3f000000u ? 0x80000000u : (0x80000000u | (b << 8));
+}
+
 // rec for the divisor b; 0 where b takes the hardware division.
 __device__ __forceinline__ unsigned div_rec(double b) {
     const unsigned hi = static_cast<unsigned>(__double2hiint(b)), lo = static_cast<unsigned>(__double2loint(b));
     const unsigned e = (hi >> 20) & 0x7ffu;
     const unsigned bt = 0x80000000u | (hi << 11) | (lo >> 21);          // mb / 2^21, rounded down
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint_as_float(0x3f800000u | ((bt >> 8) & 0x7fffffu))));
-    const unsigned rb = __float_as_uint(r);
-    const unsigned rec0 = rb >= 0x3f800000u ? 0xffffffffu : (0x80000000u | (rb << 8));
+    const unsigned rec0 = approx_bits(approx_rcp(__uint_as_float(0x3f800000u | ((bt >> 8) & 0x7fffffu))));
     const long long t = static_cast<long long>(0x8000000000000000ull - static_cast<unsigned long long>(bt) * rec0);
     const int corr = __mulhi(static_cast<int>(t >> 10), static_cast<int>(rec0 >> 1)) >> 20;
     // (rec0 + corr may pass 2^32 when mb is near 2^52)
@@ -81,7 +107,7 @@ __device__ __forceinline__ double div_by(double a, double b, unsigned rec) {
     double r = __longlong_as_double(static_cast<long long>(zero ? sign : bits));
     // (with e >= 2046 a rounding carry could reach the infinity's exponent)
     if (rec == 0u || (!zero && (static_cast<unsigned>(ea - 1) >= 2046u || static_cast<unsigned>(e - 1) >= 2045u)))
-        asm volatile("div.rn.f64 %0, %1, %2;" : "=d"(r) : "d"(a), "d"(b));   // volatile: not computed ahead of the branch
+        r = hardware_div(a, b);
     return r;
 }
 
@@ -100,12 +126,8 @@ __device__ __forceinline__ double sqrt_int(double d) {
     const unsigned long long M =
         ((static_cast<unsigned long long>((hi & 0xfffffu) | 0x100000u) << 32) | lo) << even;
     const unsigned Mt = static_cast<unsigned>(M >> 22);
-    float y;
-    asm("rsqrt.approx.ftz.f32 %0, %1;"
-        : "=f"(y)
-        : "f"(__uint_as_float(((127u + even) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29))));
-    const unsigned yb = __float_as_uint(y);
-    const unsigned Y0 = yb >= 0x3f800000u ? 0xffffffffu : (0x80000000u | (yb << 8));
+    const unsigned Y0 = approx_bits(
+        approx_rsqrt(__uint_as_float(((127u + even) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29))));
     const long long err = static_cast<long long>(0x4000000000000000ull -
                                                  static_cast<unsigned long long>(Mt) * __umulhi(Y0, Y0));
     const int corr = __mulhi(static_cast<int>(err >> 11), static_cast<int>(Y0 >> 1)) >> 19;
@@ -128,7 +150,7 @@ __device__ __forceinline__ double sqrt_int(double d) {
     S += rem > S ? 1 : 0;
     double r = __longlong_as_double(
         static_cast<long long>(static_cast<unsigned long long>((ex - even + 1023u) / 2u - 1u) << 52) + S);
-    if (ex - 1u >= 2046u) asm volatile("sqrt.rn.f64 %0, %1;" : "=d"(r) : "d"(d));
+    if (ex - 1u >= 2046u) r = hardware_sqrt(d);
     return r;
 }
 
