@@ -225,7 +225,11 @@ __device__ __forceinline__ void solve_wait(const int* flag, int want, SolveSync*
 // those, 16 right-hand sides: n = 12001 1.57 -> 0.75 ms, 32768 5.08 -> 1.95 (four: 8192 0.97 -> 0.32).
 //
 // Progress needs the cluster only: while it waits for updates that nobody has
-// taken its waiting warps take them.
+// taken its waiting warps take them over, each CTA's its own 16 rows.  With no
+// other CTA resident n = 4000 takes 22 ms and 8192 109 (16 right-hand sides; 281 and
+// 2 734 when one warp did a whole task, an element at a time).  Beside a stream
+// of matrix products that fills the chip n = 4000 takes 2.5 ms, 32768 5 (by way of
+// work items 3.5 and 9.5).
 // ---------------------------------------------------------------------------
 constexpr int kChainCtas = 8;
 constexpr int kChainThreads = 256;                           // of the products; as many fetch coefficients
@@ -234,7 +238,8 @@ constexpr int kChainNear = 4;                                // blocks before it
 constexpr int kChainNb = SolveNB<float>::value;              // 128
 constexpr int kChainRows = kChainNb / kChainCtas;            // 16: a chain CTA's rows, an urgent item's rows
 constexpr int kChainPitch = kChainNb + 4;                    // floats: 16-byte rows in distinct bank groups
-constexpr unsigned long long kChainPatience = 20000;         // ns until a waiting chain CTA takes an item
+constexpr unsigned long long kChainPatience = 20000;         // ns until a waiting chain CTA takes a task
+constexpr int kChainTaken = 256;                             // done[]: units below, taken tasks from here on
 
 // Shared memory (floats).  Chain: two sums of 16-row products, two sets of
 // coefficients, the ring of solutions, U, two V.  Task of RT rows: the sums' last
@@ -404,69 +409,117 @@ struct ChainTile {
     static_assert(KS >= 1 && KN % 4 == 0, "a share is a multiple of four terms");
 };
 
-// A task taken by a waiting warp of the chain, whose steps are all solved: from
-// global memory, in the order of the other form.
+// 16 rows of a task that the chain took over, whose steps are all solved: by one
+// warp, from global memory, in the order of the other form.  A lane has one
+// column and NCW / 2 rows, eight at a time.
 template <int NCW, int RT>
-__device__ __noinline__ void chain_task_direct(const ChainArgs& a, const ChainTask k) {
+__device__ __noinline__ void chain_unit_direct(const ChainArgs& a, int ph, int t, int rank) {
     constexpr int KS = ChainTile<NCW, RT>::KS, KN = ChainTile<NCW, RT>::KN;
-    const int r0 = chain_block(a, k.ph, k.t) * kChainNb + RT * k.part, lane = threadIdx.x & 31;
-    const int rows = min(RT, a.n - r0);
-    float* V = k.ph == 0 ? a.Y : a.X;
-    const float* Z = k.ph == 0 ? a.X : a.Y;
-    for (int e = lane; e < rows * NCW; e += 32) {
-        const int i = r0 + e / NCW, c = e % NCW;
-        float acc = 0.0f;
-        for (int ks = 0; ks < KS; ++ks) {
-            float sum = 0.0f;
-            for (int s = 0; s < k.t - kChainNear; ++s) {
-                const int c0 = chain_block(a, k.ph, s) * kChainNb;
-                float run = 0.0f;
-                for (int p = c0 + ks * KN; p < min(c0 + (ks + 1) * KN, a.n); ++p) {
-                    const float l = (a.chol && k.ph == 1) ? a.LU[idx(p, i, a.lda)] : a.LU[idx(i, p, a.lda)];
-                    run = fmaf(l, __ldcg(Z + static_cast<size_t>(p) * NCW + c), run);
-                }
-                sum += run;
-            }
-            acc += sum;
+    constexpr int J = NCW / 2 < 8 ? NCW / 2 : 8, RS = 32 / NCW;
+    const int lane = threadIdx.x & 31, c = lane % NCW, r0 = chain_block(a, ph, t) * kChainNb + rank * kChainRows;
+    const bool trans = a.chol && ph == 1;
+    const size_t rs = trans ? 1 : a.lda, ps = trans ? a.lda : 1;    // element (row, p) at rs row + ps p
+    float* V = (ph == 0 ? a.Y : a.X) + c;
+    const float* Z = (ph == 0 ? a.X : a.Y) + c;
+#pragma unroll 1
+    for (int r = r0 + lane / NCW; r < r0 + kChainRows && r0 < a.n; r += RS * J) {
+        const float* L[J];
+        float acc[J];
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            L[j] = a.LU + rs * min(r + RS * j, a.n - 1);
+            acc[j] = 0.0f;
         }
-        float* v = V + static_cast<size_t>(i) * NCW + c;
-        *v = __ldcg(v) - acc;
+#pragma unroll 1
+        for (int ks = 0; ks < KS; ++ks) {
+            float sum[J];
+#pragma unroll
+            for (int j = 0; j < J; ++j) sum[j] = 0.0f;
+#pragma unroll 1
+            for (int s = 0; s < t - kChainNear; ++s) {
+                const int p0 = chain_block(a, ph, s) * kChainNb + ks * KN, p1 = min(p0 + KN, a.n);
+                float run[J];
+#pragma unroll
+                for (int j = 0; j < J; ++j) run[j] = 0.0f;
+#pragma unroll 4
+                for (int p = p0; p < p1; ++p) {
+                    const float z = __ldcg(Z + static_cast<size_t>(p) * NCW);
+#pragma unroll
+                    for (int j = 0; j < J; ++j) run[j] = fmaf(L[j][ps * p], z, run[j]);
+                }
+#pragma unroll
+                for (int j = 0; j < J; ++j) sum[j] += run[j];
+            }
+#pragma unroll
+            for (int j = 0; j < J; ++j) acc[j] += sum[j];
+        }
+#pragma unroll
+        for (int j = 0; j < J; ++j)
+            if (r + RS * j < a.n) {
+                float* v = V + static_cast<size_t>(r + RS * j) * NCW;
+                *v = __ldcg(v) - acc[j];
+            }
     }
     __syncwarp();
     if (lane == 0) {
         __threadfence();
-        atomicAdd(a.done[k.ph] + k.t, RT / kChainRows);
+        atomicAdd(a.done[ph] + t, 1);
     }
     __syncwarp();
 }
 
-// One warp of a chain CTA: the wait for its block (phase ph, step s).
-template <int NCW, int RT>
-__device__ __forceinline__ void chain_wait(const ChainArgs& a, int ph, int s) {
-    if (s <= kChainNear) return;
-    const int total = chain_tasks(a.nblk, RT), want = kChainNb / kChainRows;
-    const volatile int* f = a.done[ph] + s;
-    for (;;) {
-        int cmd = -1;                                        // ready
-        if ((threadIdx.x & 31) == 0) {
-            const unsigned long long t0 = global_ns();
-            while (*f < want && cmd < 0) {
-                if (*static_cast<volatile int*>(&a.sy->timeout)) break;
-                if (global_ns() - t0 < kChainPatience) continue;
-                const int next = *static_cast<volatile int*>(&a.sy->next);
-                ChainTask k = chain_task(a.nblk, RT, next);
-                if (next >= total || k.ph > ph || (k.ph == ph && k.t > s)) {
-                    solve_wait(a.done[ph] + s, want, a.sy, a.wait_ns);       // taken: a bounded wait
-                    break;
-                }
-                if (atomicCAS(&a.sy->next, next, next + 1) == next) cmd = next;
-            }
-            __threadfence();
-        }
-        cmd = __shfl_sync(0xffffffffu, cmd, 0);
-        if (cmd < 0) return;
-        chain_task_direct<NCW, RT>(a, chain_task(a.nblk, RT, cmd));
+// The bounded wait for the rest of a block's units.
+__device__ __forceinline__ void chain_wait_units(const int* done, const ChainArgs& a) {
+    const volatile int* f = done;
+    const unsigned long long t0 = global_ns();
+    while ((*f & (kChainTaken - 1)) < kChainNb / kChainRows && *static_cast<volatile int*>(&a.sy->timeout) == 0) {
+        __nanosleep(32);
+        if (global_ns() - t0 > a.wait_ns) atomicExch(&a.sy->timeout, 1);
     }
+}
+
+// One warp of chain CTA `rank`: the wait for its block (phase ph, step s).
+// done[ph][s] holds the units that are up to date and, above them, a bit per task
+// of the block that the chain took over: after kChainPatience one of the eight
+// CTAs takes the next task if it is the block's, and each CTA does its own 16
+// rows of it.
+template <int NCW, int RT>
+__device__ __forceinline__ void chain_wait(const ChainArgs& a, int ph, int s, int rank) {
+    if (s <= kChainNear) return;
+    const int total = chain_tasks(a.nblk, RT), bit = kChainTaken << (rank * kChainRows / RT);
+    int* f = a.done[ph] + s;
+    bool own = false;                                        // its rows are still to be done here
+    if ((threadIdx.x & 31) == 0) {
+        const unsigned long long t0 = global_ns();
+        for (;;) {
+            const int v = *static_cast<volatile int*>(f);
+            if ((v & (kChainTaken - 1)) >= kChainNb / kChainRows || *static_cast<volatile int*>(&a.sy->timeout)) break;
+            if (v & bit) {
+                own = true;
+                break;
+            }
+            const unsigned long long t = global_ns() - t0;
+            if (t < kChainPatience) continue;
+            const int next = *static_cast<volatile int*>(&a.sy->next);
+            const ChainTask k = chain_task(a.nblk, RT, next);
+            if (next < total && k.ph == ph && k.t == s) {
+                if (atomicCAS(&a.sy->next, next, next + 1) == next) atomicAdd(f, kChainTaken << k.part);
+            } else if (t > a.wait_ns) {                      // taken by others
+                atomicExch(&a.sy->timeout, 1);
+                break;
+            } else {
+                __nanosleep(32);
+            }
+        }
+        __threadfence();
+    }
+    if (__shfl_sync(0xffffffffu, own ? 1 : 0, 0) == 0) return;
+    chain_unit_direct<NCW, RT>(a, ph, s, rank);
+    if ((threadIdx.x & 31) == 0) {
+        chain_wait_units(f, a);
+        __threadfence();
+    }
+    __syncwarp();
 }
 
 __device__ __forceinline__ void chain_mbar_init(unsigned long long* b, int count) {
@@ -551,7 +604,7 @@ __device__ __forceinline__ void chain_run(const ChainArgs& a, float* smem, int r
             if (a.inject && k == 0 && lane == 0) solve_wait(&a.sy->pad[0], 1, a.sy, a.wait_ns);   // test hook
             // (a buffer of two steps ago; the first V of the second phase is the last solution of the first)
             chain_follow(&s_prog, ph == 1 && s == 0 ? k : k - 1, a);
-            chain_wait<NCW, RT>(a, ph, s);
+            chain_wait<NCW, RT>(a, ph, s, rank);
             __syncwarp();
             const float* V = ph == 0 ? a.Y : a.X;
             for (int e = lane; e < ROWS * Q; e += 32)
