@@ -500,11 +500,17 @@ unsigned long long lu_kernel_launch_count(void);
  * Bounded device waits (no counterpart in the paper).  The library's kernels
  * wait on each other's progress in two places: the tensor-core Schur update
  * (mbarrier waits between its copy, MMA and epilogue warps) and the
- * triangular solve (a block's part waits for the blocks it depends on).  Each such wait gives up after a wall-clock deadline (default 4 s,
+ * triangular solve (a block's part waits for the blocks it depends on).  Each
+ * such wait gives up after a wall-clock deadline (default 4 s,
  * read on the device from %globaltimer); the kernel then stops taking work,
  * waits for its own copies and MMAs in flight, frees its tensor memory and
  * exits, and the call reports LU_ETIMEOUT (the factorizations through
- * *info = -LU_ETIMEOUT, the solves through their return value).
+ * *info = -LU_ETIMEOUT, the solves through their return value).  In the binary32
+ * solve the CTAs of the cluster that runs the chain also wait for one
+ * another's results, whose senders may be in such a wait: these give up after
+ * twice the deadline and one second, all together, and a CTA's warps wait for
+ * one another 64 times as long as the deadline and one second (never reached:
+ * what they wait for ends with the others).
  * ------------------------------------------------------------------------- */
 #define LU_WAIT_SITE_TC     0   /* tcgen05 Schur update (lu_gemm_lowp, the
                                    bf16 / fp8 factorization, ir_solve)          */

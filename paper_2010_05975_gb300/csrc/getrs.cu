@@ -175,15 +175,17 @@ constexpr int kSolveRhs = sizeof(T) == 8 ? 64 : 32;
 // Item list bookkeeping (device memory, zeroed before each pass).
 struct SolveSync {
     int next;          // next item to take
-    int timeout;
+    int timeout;       // 1: a wait ran out; 2: an exchange of the chain's cluster did
     int pad[2];
 };
 
 // Wait by thread 0 until *flag >= want, at most limit_ns of wall-clock time
 // (%globaltimer, read every 64 polls); a wait that runs out records the
-// timeout.  After any timeout every wait returns at once, so a broken run
+// timeout.  After any timeout every such wait returns at once, so a broken run
 // ends quickly (its results are then invalid and the host reports
-// LU_ETIMEOUT).
+// LU_ETIMEOUT).  The waits of a CTA's warps for one another, and of the
+// chain's CTAs for their exchanges, do not return then: they keep the CTA's
+// barriers in step, and end as soon as the waits that they depend on have.
 __device__ __forceinline__ void solve_wait(const int* flag, int want, SolveSync* sy, unsigned long long limit_ns) {
     const volatile int* f = flag;
     const volatile int* to = &sy->timeout;
@@ -195,7 +197,7 @@ __device__ __forceinline__ void solve_wait(const int* flag, int want, SolveSync*
             if (t0 == 0) {
                 t0 = now;
             } else if (now - t0 > limit_ns) {
-                atomicExch(&sy->timeout, 1);
+                atomicMax(&sy->timeout, 1);
                 return;
             }
         }
@@ -384,9 +386,10 @@ __device__ __forceinline__ void chain_bar_arrive(int id, int threads) {
 constexpr int kChainPair = kChainThreads + 32;       // the product warps and one other
 constexpr int kChainFed = 2 * kChainThreads + 32;    // and the fetching warps
 
-// A helper warp's wait for a counter in shared memory.  The other warps of the
-// CTA advance it after bounded waits of their own; the limit here lies far
-// beyond those.
+// A helper warp's wait for a counter in shared memory, which the other warps of the
+// CTA advance after bounded waits of their own.  It does not look at the
+// timeout: a helper that ran ahead of the others would arrive at their barriers
+// out of turn.  The limit lies beyond any that it can depend on.
 __device__ __forceinline__ void chain_follow(const volatile int* at, int want, const ChainArgs& a) {
     unsigned long long t0 = 0;
     while (*at < want) {
@@ -394,7 +397,7 @@ __device__ __forceinline__ void chain_follow(const volatile int* at, int want, c
         const unsigned long long now = global_ns();
         if (t0 == 0) t0 = now;
         else if (now - t0 > 64 * (a.wait_ns + 1000000000ull)) {
-            atomicExch(&a.sy->timeout, 1);
+            atomicMax(&a.sy->timeout, 1);
             break;
         }
     }
@@ -474,7 +477,7 @@ __device__ __forceinline__ void chain_wait_units(const int* done, const ChainArg
     const unsigned long long t0 = global_ns();
     while ((*f & (kChainTaken - 1)) < kChainNb / kChainRows && *static_cast<volatile int*>(&a.sy->timeout) == 0) {
         __nanosleep(32);
-        if (global_ns() - t0 > a.wait_ns) atomicExch(&a.sy->timeout, 1);
+        if (global_ns() - t0 > a.wait_ns) atomicMax(&a.sy->timeout, 1);
     }
 }
 
@@ -505,7 +508,7 @@ __device__ __forceinline__ void chain_wait(const ChainArgs& a, int ph, int s, in
             if (next < total && k.ph == ph && k.t == s) {
                 if (atomicCAS(&a.sy->next, next, next + 1) == next) atomicAdd(f, kChainTaken << k.part);
             } else if (t > a.wait_ns) {                      // taken by others
-                atomicExch(&a.sy->timeout, 1);
+                atomicMax(&a.sy->timeout, 1);
                 break;
             } else {
                 __nanosleep(32);
@@ -531,9 +534,11 @@ __device__ __forceinline__ void chain_mbar_expect(unsigned long long* b, unsigne
                      static_cast<unsigned>(__cvta_generic_to_shared(b))), "r"(bytes)
                  : "memory");
 }
-// The stores of all eight CTAs for one exchange are in; bounded: the time limit
-// of the other waits.
-__device__ __forceinline__ void chain_mbar_wait(unsigned long long* b, unsigned parity, const ChainArgs& a) {
+// The stores of all eight CTAs for one exchange (the copies of a stage) are in.
+// They come within the time limit of the waits that their senders may be in; past
+// that (and once another such wait has found so) they are given up: false, and
+// the chain goes through its remaining steps without exchanges.
+__device__ __forceinline__ bool chain_mbar_wait(unsigned long long* b, unsigned parity, const ChainArgs& a) {
     const unsigned at = static_cast<unsigned>(__cvta_generic_to_shared(b));
     unsigned long long t0 = 0;
     for (unsigned it = 1;; ++it) {
@@ -545,13 +550,14 @@ __device__ __forceinline__ void chain_mbar_wait(unsigned long long* b, unsigned 
             : "=r"(ok)
             : "r"(at), "r"(parity)
             : "memory");
-        if (ok) return;
+        if (ok) return true;
         if ((it & 63) == 0) {
+            if (*static_cast<volatile int*>(&a.sy->timeout) == 2) return false;
             const unsigned long long now = global_ns();
             if (t0 == 0) t0 = now;
             else if (now - t0 > 2 * a.wait_ns + 1000000000ull) {
-                atomicExch(&a.sy->timeout, 1);
-                return;
+                atomicExch(&a.sy->timeout, 2);
+                return false;
             }
         }
     }
@@ -654,38 +660,39 @@ __device__ __forceinline__ void chain_run(const ChainArgs& a, float* smem, int r
                 chain_st4(d, db, v);
             }
         };
+        bool on = true;                                      // every exchange so far has come
         for (int k = 0; k < steps; ++k) {
             const int ph = k < nblk ? 0 : 1, s = k - ph * nblk, gr = grow(k) + row;
             const float* d = Cf + (k & 1) * SET;
-            if (tid == 0) chain_mbar_expect(bars, kBytes);
+            if (tid == 0 && on) chain_mbar_expect(bars, kBytes);
             chain_bar_sync(2 + (k & 1), kChainFed);          // V and the coefficients are in
             float4 u = *reinterpret_cast<const float4*>(Vs + (k & 1) * ROWS * NCW + row * NCW + c);
             float acc[NCW / 8][4] = {};
 #pragma unroll 1
             for (int j = min(kChainNear, s); j >= 2; --j)
                 chain_product<NCW>(d + j * ROWS * CP, Zr + (s - j) % RING * NB * NCW, acc);
-            if (k >= 1) chain_mbar_wait(bars + 1, (k - 1) & 1, a);
-            if (tid == 0) chain_mbar_expect(bars + 1, kBytes);
+            if (k >= 1) on = on && chain_mbar_wait(bars + 1, (k - 1) & 1, a);
+            if (tid == 0 && on) chain_mbar_expect(bars + 1, kBytes);
             if (s >= 1) {
                 chain_product<NCW>(d + ROWS * CP, Zr + (s - 1) % RING * NB * NCW, acc);
                 chain_put<NCW>(red, acc);
                 chain_bar_sync(1, kChainThreads);
                 if (gr < a.n) u = chain_sub(u, chain_sum<NCW>(red, row, c));
             }
-            spread(Us + (rank * ROWS + row) * NCW + c, bars, u);
-            chain_mbar_wait(bars, k & 1, a);
+            if (on) spread(Us + (rank * ROWS + row) * NCW + c, bars, u);
+            on = on && chain_mbar_wait(bars, k & 1, a);
             float acd[NCW / 8][4] = {};
             chain_product<NCW>(d, Us, acd);
             chain_put<NCW>(red2, acd);
             chain_bar_sync(1, kChainThreads);
             float4 z = chain_sum<NCW>(red2, row, c);
             if (gr >= a.n) z = make_float4(0.f, 0.f, 0.f, 0.f);
-            spread(Zr + (s % RING * NB + rank * ROWS + row) * NCW + c, bars + 1, z);
+            if (on) spread(Zr + (s % RING * NB + rank * ROWS + row) * NCW + c, bars + 1, z);
             if (dup == 0 && gr < a.n)
                 *reinterpret_cast<float4*>((ph == 0 ? a.X : a.Y) + static_cast<size_t>(gr) * NCW + c) = z;
             chain_bar_arrive(4 + (k & 1), kChainPair);
         }
-        chain_mbar_wait(bars + 1, (steps - 1) & 1, a);       // (nothing is on its way here any more)
+        if (on) chain_mbar_wait(bars + 1, (steps - 1) & 1, a);   // (nothing is on its way here any more)
     }
     __syncwarp();
     chain_cluster_sync();
