@@ -935,8 +935,8 @@ __host__ __device__ inline PartsStep parts_step(int n, int nblk, int st, int sub
     return s;
 }
 
-// off[st] = items before step st, off[2 nblk] = their number; one thread, once
-// per pass width (the splits differ).
+// off[st] = items before step st, off[2 nblk] = their number, for a pass of one
+// width (the splits differ); one CTA of 256 threads, launched for every pass.
 __global__ void solve_parts_offsets_kernel(int n, int sub, int* __restrict__ off) {
     __shared__ int part[257];
     const int nblk = cdiv(n, kPartsNb), t = threadIdx.x;

@@ -91,3 +91,20 @@ def test_the_form_without_workspace_has_the_same_bits(n, nrhs, kind):
         out.append((R.cpu().numpy(), eta.cpu().numpy()))
     np.testing.assert_array_equal(out[0][0].view(np.int64), out[1][0].view(np.int64))
     np.testing.assert_array_equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("nrhs,passes", [(8, 1), (16, 1), (17, 2)])
+def test_profiled_bytes_are_those_of_the_path_taken(nrhs, passes):
+    """A is read once per 16 right-hand sides, and once for its norm, which the
+    same class counts; digits and partial sums are less than a third of it at
+    n = 2048."""
+    torch = cuda_or_fail()
+    g = lib()
+    n = 2048
+    A = torch.randn(n, n, dtype=torch.float64, device="cuda")
+    X = torch.randn(n, nrhs, dtype=torch.float64, device="cuda")
+    g.prof_begin()
+    g.lu_residual(A, X, torch.zeros_like(X))
+    torch.cuda.synchronize()
+    moved = g.prof_end()["residual"]["bytes"] - 8 * n * n
+    assert 8 * n * n * passes <= moved < 8 * n * n * passes * 4 / 3
