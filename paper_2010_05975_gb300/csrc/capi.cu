@@ -2,6 +2,7 @@
 // (Algorithm 1 on one GPU: TournPivot -> apply pivots -> FactorizeA10 ->
 // FactorizeA01 -> FactorizeA11, then the active block shrinks by w).
 #include "common.cuh"
+#include "tree_nodes.h"
 
 namespace lu {
 
@@ -45,7 +46,7 @@ struct FactorWs {
     int* counts = nullptr;
     void* a00 = nullptr;
     int* mv = nullptr;
-    size_t stride_nodes = 0;
+    size_t nodes = 0;          // that lists and counts hold
 };
 
 static void ws_free(FactorWs& ws, cudaStream_t s) {
@@ -57,9 +58,9 @@ static void ws_free(FactorWs& ws, cudaStream_t s) {
 }
 
 static int ws_alloc(FactorWs& ws, int m, int b, int h, size_t elem, cudaStream_t s) {
-    ws.stride_nodes = static_cast<size_t>(cdiv(m, h > 0 ? h : 1)) + 1;
-    bool ok = lu_malloc_async(reinterpret_cast<void**>(&ws.lists), 2 * ws.stride_nodes * b * sizeof(int), s) == cudaSuccess &&
-              lu_malloc_async(reinterpret_cast<void**>(&ws.counts), 4 * ws.stride_nodes * sizeof(int), s) == cudaSuccess &&
+    ws.nodes = tree_capacity(m, h);
+    bool ok = lu_malloc_async(reinterpret_cast<void**>(&ws.lists), ws.nodes * b * sizeof(int), s) == cudaSuccess &&
+              lu_malloc_async(reinterpret_cast<void**>(&ws.counts), 2 * ws.nodes * sizeof(int), s) == cudaSuccess &&
               lu_malloc_async(&ws.a00, static_cast<size_t>(b) * b * elem, s) == cudaSuccess &&
               lu_malloc_async(reinterpret_cast<void**>(&ws.mv), (1 + 4 * static_cast<size_t>(b)) * sizeof(int), s) == cudaSuccess;
     if (!ok) {
@@ -126,7 +127,7 @@ static int factor_loop(int m, int n, T* A, int lda, int* piv, int* info, int b, 
     const int* root = nullptr;
     if (!rc && cudaEventRecord(ev_panel, s) != cudaSuccess) rc = LU_ELAUNCH;
     if (!rc && cudaStreamWaitEvent(s2, ev_panel, 0) != cudaSuccess) rc = LU_ELAUNCH;
-    if (!rc) rc = tslu_select<T>(A, lda, m, 0, (kmax < b ? kmax : b), h, ws.lists, ws.counts, ws.stride_nodes, a00,
+    if (!rc) rc = tslu_select<T>(A, lda, m, 0, (kmax < b ? kmax : b), h, ws.lists, ws.counts, ws.nodes, a00,
                                  info, &root, s2);
     if (!rc && cudaEventRecord(ev_tslu, s2) != cudaSuccess) rc = LU_ELAUNCH;
     for (int k = 0; k < kmax && rc == 0; k += b) {
@@ -149,7 +150,7 @@ static int factor_loop(int m, int n, T* A, int lda, int* piv, int* info, int b, 
             rc = schur(A, lda, m, k, w, kn, kn + wn, s);
             if (!rc && cudaEventRecord(ev_panel, s) != cudaSuccess) rc = LU_ELAUNCH;
             if (!rc && cudaStreamWaitEvent(s2, ev_panel, 0) != cudaSuccess) rc = LU_ELAUNCH;
-            if (!rc) rc = tslu_select<T>(A, lda, m, kn, wn, h, ws.lists, ws.counts, ws.stride_nodes, a00, info,
+            if (!rc) rc = tslu_select<T>(A, lda, m, kn, wn, h, ws.lists, ws.counts, ws.nodes, a00, info,
                                          &root, s2);
             if (!rc && cudaEventRecord(ev_tslu, s2) != cudaSuccess) rc = LU_ELAUNCH;
             if (!rc) rc = schur(A, lda, m, k, w, kn + wn, n, s);
@@ -258,7 +259,7 @@ static int factor_lowp(int m, int n, float* A, int lda, int* piv, int* info, int
     const int* root = nullptr;
     if (!rc && cudaEventRecord(ev_panel, s) != cudaSuccess) rc = LU_ELAUNCH;
     if (!rc && cudaStreamWaitEvent(s2, ev_panel, 0) != cudaSuccess) rc = LU_ELAUNCH;
-    if (!rc) rc = tslu_select<float>(A, lda, m, 0, (kmax < b ? kmax : b), h, ws.lists, ws.counts, ws.stride_nodes, a00,
+    if (!rc) rc = tslu_select<float>(A, lda, m, 0, (kmax < b ? kmax : b), h, ws.lists, ws.counts, ws.nodes, a00,
                                      info, &root, s2);
     if (!rc && cudaEventRecord(ev_tslu, s2) != cudaSuccess) rc = LU_ELAUNCH;
     for (int k = 0; k < kmax && rc == 0; k += b) {
@@ -288,7 +289,7 @@ static int factor_lowp(int m, int n, float* A, int lda, int* piv, int* info, int
         rc = schur_tc_apply(A, lda, kn, kn, m - kn, wn, P, np, fp8, info, false, s);
         if (!rc && cudaEventRecord(ev_panel, s) != cudaSuccess) rc = LU_ELAUNCH;
         if (!rc && cudaStreamWaitEvent(s2, ev_panel, 0) != cudaSuccess) rc = LU_ELAUNCH;
-        if (!rc) rc = tslu_select<float>(A, lda, m, kn, wn, h, ws.lists, ws.counts, ws.stride_nodes, a00, info,
+        if (!rc) rc = tslu_select<float>(A, lda, m, kn, wn, h, ws.lists, ws.counts, ws.nodes, a00, info,
                                          &root, s2);
         if (!rc && cudaEventRecord(ev_tslu, s2) != cudaSuccess) rc = LU_ELAUNCH;
         if (!rc && np == d) {

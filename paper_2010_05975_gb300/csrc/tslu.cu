@@ -19,6 +19,7 @@
 #include "node_gepp_cluster.cuh"
 #include "node_gepp_regs.cuh"
 #include "prof.cuh"
+#include "tree_nodes.h"
 #include <cooperative_groups.h>
 #include <climits>
 
@@ -665,15 +666,16 @@ int tslu_max_cluster() {
 
 template <typename T>
 int tslu_select(const T* A, int lda, int m, int k, int w, int h, int* lists, int* counts,
-                size_t list_stride_nodes, T* a00, int* info, const int** root_list, cudaStream_t s) {
+                size_t nodes, T* a00, int* info, const int** root_list, cudaStream_t s) {
     const TsluShape sh = tslu_shape(m, k, w, h, tslu_max_cluster(), sizeof(T));
     if (int rc_ = sh.blocked == 3   ? smem_attr(tslu_tree_kernel<T>, sh.smem)
                   : sh.blocked == 1 ? smem_attr(tslu_level_kernel<T, 1>, sh.smem)
                   : sh.blocked == 2 ? smem_attr(tslu_level_kernel<T, 2>, sh.smem)
                                     : smem_attr(tslu_level_kernel<T, 0>, sh.smem))
         return rc_;
-    int* list_buf[2] = {lists, lists + list_stride_nodes * w};
-    int* cnt_buf[2] = {counts, counts + list_stride_nodes};
+    if (tree_nodes(static_cast<size_t>(sh.nsuper)) > nodes) return LU_EUNSUPPORTED;   // (ws_alloc sizes them for any k)
+    int* list_buf[2] = {lists, lists + nodes / 2 * w};
+    int* cnt_buf[2] = {counts, counts + nodes / 2};
     LevelArgs<T> args{};
     args.A = A;
     args.lda = lda;
@@ -697,10 +699,10 @@ int tslu_select(const T* A, int lda, int m, int k, int w, int h, int* lists, int
     args.child_cnt = nullptr;
     if (sh.blocked == 3) {
         // the whole tree in one launch: lists and counts level after level,
-        // arrival counts after the counts (2 list_stride_nodes each)
+        // arrival counts after the counts (`nodes` each)
         args.out_list = lists;
         args.out_cnt = counts;
-        int* arrive = counts + 2 * list_stride_nodes;
+        int* arrive = counts + nodes;
         int total = 0, rbase = 0;
         for (int k = nn; ; k = (k + 1) >> 1) {
             rbase = total;
