@@ -38,9 +38,15 @@ __host__ __device__ inline int panel_width(const Widths& t, int n) { return t.w[
 // two largest finished after 202 ms, the work of all SMs being 105 ms each.
 // There an SM's first CTA takes from the front; its second one takes from the
 // front as long as the SM's share of the whole batch's work (plus a
-// sixteenth) allows it, then from the back, the smallest, and ends when not
-// even those fit: 132 ms.
+// sixteenth and kSlackWork, below which nothing is bound by the FP64 pipes)
+// allows it, then from the back, the smallest, and ends when not even those
+// fit: 132 ms.  What a CTA takes is what one atomic addition gives it: a look at
+// the queue first decides the end, and what arrives from the front meanwhile is
+// no larger.  (With a compare-and-swap on what was looked at, the CTAs took one matrix
+// in 0.4 us between them all: 349 us for 600 of n = 16, now 112.)
 constexpr int kSmIds = 256;
+constexpr unsigned kQueueBias = 1u << 20; // both ends start here: takes past the end (one a CTA) do not wrap
+constexpr unsigned long long kSlackWork = 512;           // a matrix of order 128
 struct Queue {
     unsigned long long ends;              // next at the front (low word), end of the queue (high word)
     unsigned long long total;             // the batch's work
@@ -54,30 +60,27 @@ __host__ __device__ inline unsigned long long matrix_work(int n) {
 }
 
 // The position in `order` of the CTA's next matrix, or -1 (thread 0).
-__device__ __forceinline__ int take_front(Queue* q, int batch) {
-    const unsigned t = static_cast<unsigned>(atomicAdd(&q->ends, 1ull));
-    return t < static_cast<unsigned>(batch) ? static_cast<int>(t) : -1;
+__device__ __forceinline__ int queue_take(Queue* q, bool back) {
+    const unsigned long long e = atomicAdd(&q->ends, back ? 0xffffffff00000000ull : 1ull);
+    const unsigned f = static_cast<unsigned>(e), b = static_cast<unsigned>(e >> 32);
+    return f < b ? static_cast<int>((back ? b - 1 : f) - kQueueBias) : -1;
 }
 __device__ __forceinline__ int take_shared(Queue* q, const int* order, const int* ns, unsigned sm, bool first,
                                            unsigned long long limit) {
-    volatile unsigned long long* load = &q->load[sm];
-    for (;;) {                            // (a failed exchange means that another CTA took one)
+    bool back = false;
+    if (!first) {
+        const unsigned long long load = *reinterpret_cast<volatile unsigned long long*>(&q->load[sm]);
         const unsigned long long e = *reinterpret_cast<volatile unsigned long long*>(&q->ends);
         const unsigned f = static_cast<unsigned>(e), b = static_cast<unsigned>(e >> 32);
         if (f >= b) return -1;
-        unsigned t = f;
-        unsigned long long w = matrix_work(ns[order[f]]);
-        if (!first && *load + w > limit) {
-            t = b - 1;
-            w = matrix_work(ns[order[t]]);
-            if (*load + w > limit) return -1;
-        }
-        const unsigned long long to = t == f ? e + 1 : e - (1ull << 32);
-        if (atomicCAS(&q->ends, e, to) == e) {
-            atomicAdd(&q->load[sm], w);
-            return static_cast<int>(t);
+        if (load + matrix_work(ns[order[f - kQueueBias]]) > limit) {
+            if (load + matrix_work(ns[order[b - 1 - kQueueBias]]) > limit) return -1;
+            back = true;
         }
     }
+    const int t = queue_take(q, back);
+    if (t >= 0) atomicAdd(&q->load[sm], matrix_work(ns[order[t]]));
+    return t;
 }
 
 template <typename T>
@@ -93,7 +96,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2)
         asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
         smid %= kSmIds;
         first = atomicAdd(&q->slot[smid], 1) == 0;
-        limit = q->total / sms + q->total / sms / 16;
+        limit = q->total / sms + q->total / sms / 16 + kSlackWork;
         // a later CTA of the SM waits (a fraction of a millisecond at most)
         // until the first one has taken its matrix
         for (int i = 0; !first && i < 4096; ++i) {
@@ -106,7 +109,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2)
     }
     for (;;) {
         if (threadIdx.x == 0)
-            sm.next = sizeof(T) == 4 ? take_front(q, batch) : take_shared(q, order, ns, smid, first, limit);
+            sm.next = sizeof(T) == 4 ? queue_take(q, false) : take_shared(q, order, ns, smid, first, limit);
         __syncthreads();
         const int t = sm.next;
         __syncthreads();
@@ -183,7 +186,7 @@ __global__ void __launch_bounds__(1024) size_scan_kernel(int batch, int* __restr
                               static_cast<unsigned long long>(b) * matrix_work(kMaxN - i0 - 1);
     for (int o = 16; o > 0; o >>= 1) work += __shfl_xor_sync(0xffffffffu, work, o);
     if (lane == 0 && work != 0) atomicAdd(&q->total, work);
-    if (tid == 0) q->ends = static_cast<unsigned long long>(batch) << 32;
+    if (tid == 0) q->ends = (static_cast<unsigned long long>(kQueueBias + static_cast<unsigned>(batch)) << 32) | kQueueBias;
 }
 __global__ void size_scatter_kernel(int batch, const int* __restrict__ ns, int* __restrict__ hist,
                                     int* __restrict__ order) {
