@@ -172,10 +172,11 @@ __global__ void __launch_bounds__(4 * SolveNB<T>::value) invert_diag_kernel(int 
 template <typename T>
 constexpr int kSolveRhs = sizeof(T) == 8 ? 64 : 32;
 
-// Item list bookkeeping (device memory, zeroed before each pass).
+// Item list bookkeeping (device memory, zeroed before each pass but for timeout,
+// which a call's passes share and the host reads once, after the last).
 struct SolveSync {
-    int next;          // next item to take
     int timeout;       // 1: a wait ran out; 2: an exchange of the chain's cluster did
+    int next;          // next item to take
     int pad[2];
 };
 
@@ -1338,7 +1339,8 @@ int solve_plan_apply(const SolvePlan<T>& p, int nrhs, T* B, int ldb, cudaStream_
         const int w = nc <= 8 ? 8 : nc <= 16 ? 16 : nc <= 32 ? 32 : 64;
         const long long tot = static_cast<long long>(n) * w;
         const int gblocks = static_cast<int>(tot / 256 + 1 < 4096 ? tot / 256 + 1 : 4096);
-        if (cudaMemsetAsync(ws, 0, flags, s) != cudaSuccess) {
+        const size_t kept = c0 > 0 ? offsetof(SolveSync, next) : 0;
+        if (cudaMemsetAsync(static_cast<unsigned char*>(ws) + kept, 0, flags - kept, s) != cudaSuccess) {
             rc = LU_ELAUNCH;
             break;
         }
@@ -1370,14 +1372,10 @@ int solve_plan_apply(const SolvePlan<T>& p, int nrhs, T* B, int ldb, cudaStream_
             rc = LU_ELAUNCH;
             break;
         }
-        int to = 0;
-        if (cudaMemcpyAsync(&to, &sy->timeout, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-            cudaStreamSynchronize(s) != cudaSuccess) {
-            rc = LU_ELAUNCH;
-            break;
-        }
-        timeout |= to;
     }
+    if (!rc && (cudaMemcpyAsync(&timeout, &sy->timeout, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+                cudaStreamSynchronize(s) != cudaSuccess))
+        rc = LU_ELAUNCH;
     if (!rc && timeout) rc = LU_ETIMEOUT;
     cudaFreeAsync(ws, s);
     return rc;
