@@ -43,7 +43,7 @@ __host__ __device__ inline int panel_width(const Widths& t, int n) { return t.w[
 // fit: 132 ms.  What a CTA takes is what one atomic addition gives it: a look at
 // the queue first decides the end, and what arrives from the front meanwhile is
 // no larger.  (With a compare-and-swap on what was looked at, the CTAs took one matrix
-// in 0.4 us between them all: 349 us for 600 of n = 16, now 112.)
+// in 0.4 us between them all: 349 us for 600 of n = 16, now 94.)
 constexpr int kSmIds = 256;
 constexpr unsigned kQueueBias = 1u << 20; // both ends start here: takes past the end (one a CTA) do not wrap
 constexpr unsigned long long kSlackWork = 512;           // a matrix of order 128
